@@ -70,10 +70,10 @@ TRAFFIC = {"files": ["paper_2006_02501_gb300/csrc/pair_fix.cu",
                      "paper_2006_02501_gb300/csrc/fix_sum.cuh",
                      "paper_2006_02501_gb300/csrc/pair_sym.cuh"],
            "sha256": [
-               "a9a059cd831b190a0cdcf5f23c8a5bd892f92caf6378eb4e8f1f4b45c4242467",
+               "b7ce046add8aefc81272fc52e453b8537459cbd537405a00f7c1b2623ba54885",
                "13be02ddd079262f0c64645f723e2ee2e12df53b9da4ce333bb33ee4478f1735",
                "ae11452433433fc22ea3655564a16804e5ffde57e751852eeb61a046355aee89",
-               "c84ad924123b9906c6ff937593d09f5bdd604e0c218208f969584102545afa4a"],
+               "1f0598f969a1334d8da9f876f87927fc5e369136c5e96fd84acba341d9b6ca6c"],
            # profiles/k_pair_fix_sym_disc_order8.md: 15.63 MB read + 39.19 MB written
            "bytes_per_launch": 15.63e6 + 39.19e6,
            # the same file: ALU-pipe thread instructions per unordered pair (ncu, 16385 bodies)

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kSymR * sym64_rows, 1) k_pair_fp64_sym(SymArgs
                 for (int k = 0; k <= P; ++k)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) accj[k][c] = jt == 0 ? 0.0 : accs[3 * k + c][js * 32 + lane];
-                ring_tile<P, kH>(a, (int64_t)J * kSymR + js * 32, lane, ri, gmi, acci, accj, wm);
+                ring_tile<P, kH>(a, (int64_t)J * kSymR + js * 32, lane, ib < a.N, ri, gmi, acci, accj, wm);
 #pragma unroll
                 for (int k = 0; k <= P; ++k)
 #pragma unroll

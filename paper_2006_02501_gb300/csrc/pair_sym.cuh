@@ -245,7 +245,7 @@ __device__ __forceinline__ void rotate(double (&r)[P + 1][3], double &gm, int sr
 }
 
 // Subtiles [t0, t1) of the diagonal block of row I in FP64: ordered pairs into the
-// i-side sums only.
+// i-side sums only.  kH: a padding body counts for no pair, however close it is.
 template <int P, bool kH>
 __device__ __forceinline__ void ring_diag(const SymArgs<P> &a, int I, int t0, int t1, int w, int lane,
                                           const double (&ri)[P + 1][3], double gmi, double (&acci)[P + 1][3],
@@ -255,6 +255,8 @@ __device__ __forceinline__ void ring_diag(const SymArgs<P> &a, int I, int t0, in
     for (int js = t0; js < t1; ++js) {
         double rj[P + 1][3], gmj;
         load_body<P>(a, (int64_t)I * kSymR + js * 32 + lane, rj, gmj);
+        [[maybe_unused]] const int64_t n_real =
+            (int64_t)I * kSymR + w * 32 + lane < a.N ? a.N - ((int64_t)I * kSymR + js * 32) : 0;
         for (int t = 0; t < 32; ++t) {
             const bool self = js == w && t == 0;
             double r[P + 1][3];
@@ -270,7 +272,8 @@ __device__ __forceinline__ void ring_diag(const SymArgs<P> &a, int I, int t0, in
             const double S = rinv * sinv;
             const double mS = wi * S;
             if constexpr (kH) {
-                const unsigned long long wb = self ? 0ull : (unsigned long long)__double_as_longlong((gmi + gmj) * S);
+                const bool real = !self && ((lane + t) & 31) < n_real;
+                const unsigned long long wb = real ? (unsigned long long)__double_as_longlong((gmi + gmj) * S) : 0ull;
                 wm = wb > wm ? wb : wm;
             }
             pair_odd_terms<P, double>(r, sinv, [&](int k, int c, double B) {
@@ -283,11 +286,13 @@ __device__ __forceinline__ void ring_diag(const SymArgs<P> &a, int I, int t0, in
 
 // One 32-body j-subtile (bodies jb .. jb + 31) against the warp's i-bodies in
 // FP64: a ring in which the j-body and its j-side sums accj travel lane by lane.
+// real_i: this thread's i-body is no padding.
 template <int P, bool kH>
-__device__ __forceinline__ void ring_tile(const SymArgs<P> &a, int64_t jb, int lane, const double (&ri)[P + 1][3],
-                                          double gmi, double (&acci)[P + 1][3], double (&accj)[P + 1][3],
-                                          unsigned long long &wm)
+__device__ __forceinline__ void ring_tile(const SymArgs<P> &a, int64_t jb, int lane, bool real_i,
+                                          const double (&ri)[P + 1][3], double gmi, double (&acci)[P + 1][3],
+                                          double (&accj)[P + 1][3], unsigned long long &wm)
 {
+    [[maybe_unused]] const int64_t n_real = real_i ? a.N - jb : 0;      // j-lanes that hold bodies
     const int src = (lane + 1) & 31;      // after t passes lane l holds j-lane (l + t) mod 32
     double rj[P + 1][3], gmj;
     load_body<P>(a, jb + lane, rj, gmj);
@@ -303,7 +308,8 @@ __device__ __forceinline__ void ring_tile(const SymArgs<P> &a, int64_t jb, int l
         const double S = rinv * sinv;
         const double wi = gmj * S, wj = gmi * S;
         if constexpr (kH) {
-            const unsigned long long wb = (unsigned long long)__double_as_longlong(wi + wj);
+            const unsigned long long wb =
+                ((lane + t) & 31) < n_real ? (unsigned long long)__double_as_longlong(wi + wj) : 0ull;
             wm = wb > wm ? wb : wm;
         }
         pair_odd_terms<P, double>(r, sinv, [&](int k, int c, double B) {
