@@ -57,7 +57,7 @@ __device__ __forceinline__ void stage(bf16 (*dst)[cols + kPad16], const bf16 *__
             if (vec && c + 8 <= cmax) {
                 v = *reinterpret_cast<const uint4 *>(q);
             } else {
-                bf16 w[8];
+                __align__(16) bf16 w[8];           // read as one 16-byte word below
 #pragma unroll
                 for (int k = 0; k < 8; ++k) w[k] = c + k < cmax ? q[k] : __float2bfloat16(0.0f);
                 v = *reinterpret_cast<const uint4 *>(w);
