@@ -39,7 +39,8 @@ __device__ __forceinline__ float dsilu(float z)
 enum { kStore = 0,       // c = sum
        kBias = 1,        // c = sum + bias
        kBiasSilu = 2,    // c = z = sum + bias, h = bf16(silu(z))
-       kDsilu = 3 };     // h = bf16(sum * silu'(c)), c read
+       kDsilu = 3,       // h = bf16(sum * silu'(c)), c read
+       kSilu = 4 };      // h = bf16(silu(sum + bias)): inference, which reads no z again
 
 // Rows x cols bf16 tile src[r * ld + c] to shared memory [rows][cols + kPad16], zero
 // outside rmax x cmax.  128 threads; vec: 16-byte loads (base and ld allow them).
@@ -161,8 +162,8 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K, const bf
                     h[e] = __float2bfloat16(acc[i][j][q] * dsilu(c[e]));
                 } else {
                     const float z = EPI == kStore ? acc[i][j][q] : acc[i][j][q] + bias[n];
-                    c[e] = z;
-                    if (EPI == kBiasSilu) h[e] = __float2bfloat16(silu(z));
+                    if (EPI != kSilu) c[e] = z;
+                    if (EPI == kBiasSilu || EPI == kSilu) h[e] = __float2bfloat16(silu(z));
                 }
             }
 }
@@ -393,7 +394,8 @@ struct mh_mlp {
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     bf16 *p16 = nullptr;
     int64_t t = 0;
-    int64_t cap = 0;                 // rows of the workspace
+    int64_t cap = 0;                 // rows of X16, H1, H2: all that inference needs
+    int64_t cap_train = 0;           // rows of the other buffers
     bf16 *X16 = nullptr, *H1 = nullptr, *H2 = nullptr, *dY16 = nullptr, *dZ2 = nullptr, *dZ1 = nullptr;
     float *Z1 = nullptr, *Z2 = nullptr, *Y = nullptr, *T = nullptr;
     double *lpart = nullptr, *lsum = nullptr;
@@ -404,54 +406,73 @@ struct mh_mlp {
 
 namespace {
 
+template <typename T>
+void drop(T *&p)
+{
+    if (p) cudaFree(p);
+    p = nullptr;
+}
+
+void free_train(mh_mlp *n)
+{
+    drop(n->dY16); drop(n->dZ2); drop(n->dZ1); drop(n->Z1); drop(n->Z2); drop(n->Y); drop(n->T);
+    drop(n->lpart); drop(n->lsum); drop(n->gpart);
+    n->cap_train = 0;
+}
+
 void free_ws(mh_mlp *n)
 {
-    void *ptrs[] = {n->X16, n->H1, n->H2, n->dY16, n->dZ2, n->dZ1, n->Z1, n->Z2, n->Y, n->T, n->lpart, n->lsum, n->gpart};
-    for (void *q : ptrs)
-        if (q) cudaFree(q);
-    n->X16 = n->H1 = n->H2 = n->dY16 = n->dZ2 = n->dZ1 = nullptr;
-    n->Z1 = n->Z2 = n->Y = n->T = n->gpart = nullptr;
-    n->lpart = n->lsum = nullptr;
+    free_train(n);
+    drop(n->X16); drop(n->H1); drop(n->H2);
     n->cap = 0;
 }
 
-int ensure_ws(mh_mlp *n, int64_t rows, cudaStream_t st)
+// Workspace of a pass over `rows` rows: inference, or with the gradient's buffers too.
+int ensure_ws(mh_mlp *n, int64_t rows, bool train, cudaStream_t st)
 {
-    if (rows <= n->cap) return MH_OK;
-    MH_CUDA(cudaStreamSynchronize(st));
-    free_ws(n);
     const int64_t H = n->H;
-    MH_CUDA(cudaMalloc((void **)&n->X16, rows * pad8(n->n_in) * sizeof(bf16)));
-    MH_CUDA(cudaMalloc((void **)&n->H1, rows * H * sizeof(bf16)));
-    MH_CUDA(cudaMalloc((void **)&n->H2, rows * H * sizeof(bf16)));
-    MH_CUDA(cudaMalloc((void **)&n->dY16, rows * pad8(n->n_out) * sizeof(bf16)));
-    MH_CUDA(cudaMalloc((void **)&n->dZ2, rows * H * sizeof(bf16)));
-    MH_CUDA(cudaMalloc((void **)&n->dZ1, rows * H * sizeof(bf16)));
-    MH_CUDA(cudaMalloc((void **)&n->Z1, rows * H * sizeof(float)));
-    MH_CUDA(cudaMalloc((void **)&n->Z2, rows * H * sizeof(float)));
-    MH_CUDA(cudaMalloc((void **)&n->Y, rows * n->n_out * sizeof(float)));
-    MH_CUDA(cudaMalloc((void **)&n->T, rows * n->n_out * sizeof(float)));
-    const int64_t gp = (int64_t)split_parts(rows) * std::max(n->H, n->n_out);
-    MH_CUDA(cudaMalloc((void **)&n->gpart, gp * sizeof(float)));
-    MH_CUDA(cudaMalloc((void **)&n->lpart, (nb(rows * n->n_out) + 1) * sizeof(double)));
-    MH_CUDA(cudaMalloc((void **)&n->lsum, sizeof(double)));
-    // the padding columns of X16 and dY16 stay zero
-    MH_CUDA(cudaMemsetAsync(n->X16, 0, rows * pad8(n->n_in) * sizeof(bf16), st));
-    MH_CUDA(cudaMemsetAsync(n->dY16, 0, rows * pad8(n->n_out) * sizeof(bf16), st));
-    n->cap = rows;
+    if (rows > n->cap) {
+        MH_CUDA(cudaStreamSynchronize(st));
+        drop(n->X16); drop(n->H1); drop(n->H2);
+        n->cap = 0;
+        MH_CUDA(cudaMalloc((void **)&n->X16, rows * pad8(n->n_in) * sizeof(bf16)));
+        MH_CUDA(cudaMalloc((void **)&n->H1, rows * H * sizeof(bf16)));
+        MH_CUDA(cudaMalloc((void **)&n->H2, rows * H * sizeof(bf16)));
+        // the padding columns of X16 (and dY16) stay zero
+        MH_CUDA(cudaMemsetAsync(n->X16, 0, rows * pad8(n->n_in) * sizeof(bf16), st));
+        n->cap = rows;
+    }
+    if (train && rows > n->cap_train) {
+        MH_CUDA(cudaStreamSynchronize(st));
+        free_train(n);
+        MH_CUDA(cudaMalloc((void **)&n->dY16, rows * pad8(n->n_out) * sizeof(bf16)));
+        MH_CUDA(cudaMalloc((void **)&n->dZ2, rows * H * sizeof(bf16)));
+        MH_CUDA(cudaMalloc((void **)&n->dZ1, rows * H * sizeof(bf16)));
+        MH_CUDA(cudaMalloc((void **)&n->Z1, rows * H * sizeof(float)));
+        MH_CUDA(cudaMalloc((void **)&n->Z2, rows * H * sizeof(float)));
+        MH_CUDA(cudaMalloc((void **)&n->Y, rows * n->n_out * sizeof(float)));
+        MH_CUDA(cudaMalloc((void **)&n->T, rows * n->n_out * sizeof(float)));
+        const int64_t gp = (int64_t)split_parts(rows) * std::max(n->H, n->n_out);
+        MH_CUDA(cudaMalloc((void **)&n->gpart, gp * sizeof(float)));
+        MH_CUDA(cudaMalloc((void **)&n->lpart, (nb(rows * n->n_out) + 1) * sizeof(double)));
+        MH_CUDA(cudaMalloc((void **)&n->lsum, sizeof(double)));
+        MH_CUDA(cudaMemsetAsync(n->dY16, 0, rows * pad8(n->n_out) * sizeof(bf16), st));
+        n->cap_train = rows;
+    }
     return MH_OK;
 }
 
-// Forward over rows already gathered into X16; Y (fp32) receives the outputs.
+// Forward over rows already gathered into X16; Y (fp32) receives the outputs.  EPI:
+// kBiasSilu keeps the pre-activations Z1, Z2 for the gradient, kSilu does not.
+template <int EPI>
 int forward_ws(mh_mlp *n, int64_t B, float *Y, cudaStream_t st)
 {
     const int H = n->H;
     const bf16 *W1 = n->p16 + n->oW1, *W2 = n->p16 + n->oW2, *W3 = n->p16 + n->oW3;
-    if (int rc = gemm<false, true, kBiasSilu>((int)B, H, n->n_in, n->X16, pad8(n->n_in), W1, n->n_in, n->Z1, H, st,
-                                              n->p + n->ob1, n->H1))
+    if (int rc = gemm<false, true, EPI>((int)B, H, n->n_in, n->X16, pad8(n->n_in), W1, n->n_in, n->Z1, H, st,
+                                        n->p + n->ob1, n->H1))
         return rc;
-    if (int rc = gemm<false, true, kBiasSilu>((int)B, H, H, n->H1, H, W2, H, n->Z2, H, st, n->p + n->ob2, n->H2))
-        return rc;
+    if (int rc = gemm<false, true, EPI>((int)B, H, H, n->H1, H, W2, H, n->Z2, H, st, n->p + n->ob2, n->H2)) return rc;
     return gemm<false, true, kBias>((int)B, n->n_out, H, n->H2, H, W3, H, Y, n->n_out, st, n->p + n->ob3);
 }
 
@@ -510,14 +531,16 @@ namespace mh {
 // Inference for the learned predictor (learned.cu): Y[n x n_out] from X[n x n_in] (fp32, device).
 int mlp_infer(mh_mlp *n, const float *X, float *Y, int64_t rows, cudaStream_t st)
 {
-    const int64_t chunk = n->H <= 128 ? 1 << 18 : 1 << 16;     // rows per pass: the workspace stays below 1 GB
-    if (int rc = ensure_ws(n, std::min(rows, chunk), st)) return rc;
+    // rows per pass: 256 MB of X16, H1 and H2 (H = 128: 2^18 rows in 147 MB), whole tiles
+    const int64_t row_bytes = (int64_t)sizeof(bf16) * (pad8(n->n_in) + 2 * n->H);
+    const int64_t chunk = std::min<int64_t>(1 << 18, (256ll << 20) / row_bytes / kTM * kTM);
+    if (int rc = ensure_ws(n, std::min(rows, chunk), false, st)) return rc;
     for (int64_t r0 = 0; r0 < rows; r0 += chunk) {
         const int64_t B = std::min(chunk, rows - r0);
         k_gather<<<nb(B * n->n_in), 256, 0, st>>>(B, n->n_in, X + r0 * n->n_in, nullptr, n->X16, pad8(n->n_in),
                                                        nullptr);
         MH_LAUNCHED("k_gather");
-        if (int rc = forward_ws(n, B, Y + r0 * n->n_out, st)) return rc;
+        if (int rc = forward_ws<kSilu>(n, B, Y + r0 * n->n_out, st)) return rc;
     }
     return MH_OK;
 }
@@ -639,12 +662,12 @@ int mh_mlp_loss_grad(mh_mlp *n, const float *x, const float *t, int64_t rows, do
     if (int rc = check_net(n)) return rc;
     if (!x || !t || rows < 1 || rows > (1 << 24)) { set_error("mh_mlp_loss_grad: device x, t and 1 <= rows <= 2^24"); return MH_EINVAL; }
     cudaStream_t st = (cudaStream_t)stream;
-    if (int rc = ensure_ws(n, rows, st)) return rc;
+    if (int rc = ensure_ws(n, rows, true, st)) return rc;
     k_gather<<<nb(rows * n->n_in), 256, 0, st>>>(rows, n->n_in, x, nullptr, n->X16, pad8(n->n_in), nullptr);
     MH_LAUNCHED("k_gather");
     k_gather<<<nb(rows * n->n_out), 256, 0, st>>>(rows, n->n_out, t, nullptr, nullptr, 0, n->T);
     MH_LAUNCHED("k_gather");
-    if (int rc = forward_ws(n, rows, n->Y, st)) return rc;
+    if (int rc = forward_ws<kBiasSilu>(n, rows, n->Y, st)) return rc;
     if (int rc = backward_ws(n, rows, st)) return rc;
     double ls = 0.0;
     MH_CUDA(cudaMemcpyAsync(&ls, n->lsum, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -664,7 +687,7 @@ int mh_mlp_train(mh_mlp *n, const float *x, const float *t, int64_t rows, int ep
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t B = std::min<int64_t>(batch, rows);
-    if (int rc = ensure_ws(n, B, st)) return rc;
+    if (int rc = ensure_ws(n, B, true, st)) return rc;
     if (rows > n->idx_cap) {
         MH_CUDA(cudaStreamSynchronize(st));
         if (n->idx) cudaFree(n->idx);
@@ -686,7 +709,7 @@ int mh_mlp_train(mh_mlp *n, const float *x, const float *t, int64_t rows, int ep
             MH_LAUNCHED("k_gather");
             k_gather<<<nb(B * n->n_out), 256, 0, st>>>(B, n->n_out, t, n->idx + r0, nullptr, 0, n->T);
             MH_LAUNCHED("k_gather");
-            if (int rc = forward_ws(n, B, n->Y, st)) return rc;
+            if (int rc = forward_ws<kBiasSilu>(n, B, n->Y, st)) return rc;
             if (int rc = backward_ws(n, B, st)) return rc;
             n->t += 1;
             const float c1 = 1.0f - std::pow(0.9f, (float)n->t), c2 = 1.0f - std::pow(0.999f, (float)n->t);
