@@ -70,14 +70,14 @@ TRAFFIC = {"files": ["paper_2006_02501_gb300/csrc/pair_fix.cu",
                      "paper_2006_02501_gb300/csrc/fix_sum.cuh",
                      "paper_2006_02501_gb300/csrc/pair_sym.cuh"],
            "sha256": [
-               "b7ce046add8aefc81272fc52e453b8537459cbd537405a00f7c1b2623ba54885",
-               "13be02ddd079262f0c64645f723e2ee2e12df53b9da4ce333bb33ee4478f1735",
-               "ae11452433433fc22ea3655564a16804e5ffde57e751852eeb61a046355aee89",
+               "7d479842edd11e0c7ccca49b62491923e2bfb2f01cef41efef89ba2b6c20e5b8",
+               "c802ddbf2bc01bbe166b68cc004187b2551ec183e6bee6cd6593fc8650998fd6",
+               "d8ec6193aab9c24134d5972007fc7963475e8f2ecac408a8e0f0a8549176ff7e",
                "1f0598f969a1334d8da9f876f87927fc5e369136c5e96fd84acba341d9b6ca6c"],
-           # profiles/k_pair_fix_sym_disc_order8.md: 15.63 MB read + 39.19 MB written
-           "bytes_per_launch": 15.63e6 + 39.19e6,
+           # profiles/k_pair_fix_sym_disc_order8.md: 16.30 MB read + 40.29 MB written
+           "bytes_per_launch": 16.30e6 + 40.29e6,
            # the same file: ALU-pipe thread instructions per unordered pair (ncu, 16385 bodies)
-           "alu_instr_per_unordered_pair": 678.0}
+           "alu_instr_per_unordered_pair": 832.0}
 
 
 # FP64 instructions per pair interaction (ordered pair) of the double-double

@@ -17,11 +17,17 @@
 // the last term (below 1/4 unit of a result of up to 2^58) is dropped.
 //
 // Inputs.  Every component of x, v, a, a-dot of a body is a 96-bit two's
-// complement integer on one grid per row (x, v, a or a-dot) for the whole
+// complement integer on a grid per row (x, v, a or a-dot) for the whole
 // system: unit 2^(E-91), E the exponent of the largest component.  An FP64 value
 // down to 2^-38 of the largest is on the grid exactly; systems with a wider
 // range of magnitudes are evaluated in FP64 (the caller's rule).  Differences
-// are then exact, with one exponent per difference vector from its leading bit.
+// are then exact.
+//
+// The components of a vector share an exponent, from the leading bit of the largest,
+// so a small one keeps fewer bits than it would in FP64.  The flattest axis of a
+// system (a disc's), which the caller makes the third component, therefore has grids,
+// exponents and sums of its own (Fx3::e[1]): only dot products meet both.  What the
+// other two lack between them is the caller's rule again.
 //
 // Pair derivatives (Dittmann 2020, Section 3, intro), with S = s^(-3/2),
 // s = r.r + eps^2, in Leibniz form A^(k) / (G m S) = sum C(k, n) c_n r^(k-n),
@@ -148,13 +154,15 @@ MH_HD int fx_norm(long long &v)
     return n;
 }
 
-// Three components of a difference, 96-bit two's complement each (w[c] = low,
-// middle, high word, |value| < 2^93): mantissas and exponent, value =
-// M 2^(e-61) with unit 2^(E-91) of the words.
+// A vector: mantissas, and exponents of the first two components together and of the
+// third, value = M 2^(e-61).
 struct Fx3 {
     Fx c[3];
-    int e;
+    int e[2];
 };
+MH_HD constexpr int fx_group(int c) { return c == 2; }
+// components of group g: [fx_first(g), fx_first(g + 1))
+MH_HD constexpr int fx_first(int g) { return g == 0 ? 0 : g + 1; }
 
 MH_HD void sub96(const unsigned (&a)[3], const unsigned (&b)[3], unsigned (&d)[3])
 {
@@ -171,58 +179,72 @@ MH_HD void sub96(const unsigned (&a)[3], const unsigned (&b)[3], unsigned (&d)[3
 #endif
 }
 
-// Bits above 1 mark changes between neighbouring bits of a high word: the
-// leading one is one above the largest component's leading bit.
-MH_HD unsigned fold3(const unsigned (&d)[3][3])
-{
-    return (d[0][2] ^ d[0][2] + d[0][2]) | (d[1][2] ^ d[1][2] + d[1][2]) | (d[2][2] ^ d[2][2] + d[2][2]);
-}
+// Bits above 1 mark changes between neighbouring bits of a high word: the leading one
+// of the two components' (or the one's) is one above the largest's leading bit.
+MH_HD unsigned fold1(unsigned h) { return h ^ (h + h); }
 
-MH_HD Fx3 fx_diff(const unsigned (&a)[3][3], const unsigned (&b)[3][3], int E)
+// A difference of 96-bit two's complement components (w[c] = low, middle, high word,
+// |value| < 2^93), units 2^(E-91) of the first two and 2^(Ez-91) of the third.
+MH_HD Fx3 fx_diff(const unsigned (&a)[3][3], const unsigned (&b)[3][3], int E, int Ez)
 {
     unsigned d[3][3];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
     for (int c = 0; c < 3; ++c) sub96(a[c], b[c], d[c]);
-    unsigned t = fold3(d);
     Fx3 r;
-    r.e = E + 2;
-    // a difference far below the largest component: 29 bits at a time (the high
-    // words are pure sign, so 29 more bits fit)
-    for (int k = 0; k < 3 && t < 2; ++k) {
-        for (int c = 0; c < 3; ++c) {
-            d[c][2] = shl32(d[c][1], d[c][2], 29);
-            d[c][1] = shl32(d[c][0], d[c][1], 29);
-            d[c][0] <<= 29;
-        }
-        r.e -= 29;
-        t = fold3(d);
-    }
-    const int n = imin(clz32(t), 31) - 2;
-    r.e -= n;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-    for (int c = 0; c < 3; ++c) {
-        const unsigned h = shl32(d[c][1], d[c][2], n), l = shl32(d[c][0], d[c][1], n);
-        r.c[c] = Fx{(int)h + (int)(l >> 31), (int)l};
+    for (int g = 0; g < 2; ++g) {
+        auto fold = [&] { return g ? fold1(d[2][2]) : fold1(d[0][2]) | fold1(d[1][2]); };
+        unsigned t = fold();
+        int e = (g ? Ez : E) + 2;
+        // a difference far below the largest component: 29 bits at a time (the high
+        // words are pure sign, so 29 more bits fit)
+        for (int k = 0; k < 3 && t < 2; ++k) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+            for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
+                d[c][2] = shl32(d[c][1], d[c][2], 29);
+                d[c][1] = shl32(d[c][0], d[c][1], 29);
+                d[c][0] <<= 29;
+            }
+            e -= 29;
+            t = fold();
+        }
+        const int n = imin(clz32(t), 31) - 2;
+        r.e[g] = e - n;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
+            const unsigned h = shl32(d[c][1], d[c][2], n), l = shl32(d[c][0], d[c][1], n);
+            r.c[c] = Fx{(int)h + (int)(l >> 31), (int)l};
+        }
     }
     return r;
 }
 
-// Three components v 2^(e-58) to 2^60 <= max |M| <= 2^61 (or |v| < 2^32 shifted by 29).
-MH_HD Fx3 fx_norm3(const long long (&v)[3], int e)
+// Components v 2^(e-58) to 2^60 <= |M| <= 2^61 of the group's largest (or |v| < 2^32
+// shifted by 29).
+MH_HD Fx3 fx_norm3(const long long (&v)[3], const int (&e)[2])
 {
-    const unsigned h0 = (unsigned)(v[0] >> 32), h1 = (unsigned)(v[1] >> 32), h2 = (unsigned)(v[2] >> 32);
-    const unsigned t = (h0 ^ h0 + h0) | (h1 ^ h1 + h1) | (h2 ^ h2 + h2);
-    const int n = imin(clz32(t), 31) - 2;
     Fx3 r;
-    r.e = e + 3 - n;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-    for (int c = 0; c < 3; ++c) r.c[c] = fx((long long)((unsigned long long)v[c] << n));
+    for (int g = 0; g < 2; ++g) {
+        const unsigned t = g ? fold1((unsigned)(v[2] >> 32))
+                             : fold1((unsigned)(v[0] >> 32)) | fold1((unsigned)(v[1] >> 32));
+        const int n = imin(clz32(t), 31) - 2;
+        r.e[g] = e[g] + 3 - n;
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = fx_first(g); c < fx_first(g + 1); ++c) r.c[c] = fx((long long)((unsigned long long)v[c] << n));
+    }
     return r;
 }
 
@@ -231,31 +253,40 @@ MH_HD long long fx_val(Fx a)
     return (long long)((unsigned long long)(unsigned)(a.h + (a.l >> 31)) << 32 | (unsigned)a.l);
 }
 
-// value c 2^(e-61)-scaled vector shifted right by n
-MH_HD FxSum fx_dot(const Fx3 &a, const Fx3 &b)
+// a.b as v[0] 2^(e[0]-58) + v[1] 2^(e[1]-58), |v[0]| <= 2^59, |v[1]| <= 2^58.
+struct FxDot {
+    long long v[2];
+    int e[2];
+};
+
+MH_HD FxDot fx_dot(const Fx3 &a, const Fx3 &b)
 {
     FxSum s = fx_mul(a.c[0], b.c[0]);
     fx_add(s, a.c[1], b.c[1]);
-    fx_add(s, a.c[2], b.c[2]);
-    return s;
+    return FxDot{{fx_get(s), fx_get(fx_mul(a.c[2], b.c[2]))}, {a.e[0] + b.e[0], a.e[1] + b.e[1]}};
 }
 
-MH_HD FxSum fx_dot_self(const Fx3 &a)
+MH_HD FxDot fx_dot_self(const Fx3 &a)
 {
     FxSum s = fx_sqr(a.c[0]);
     fx_add_sqr(s, a.c[1]);
-    fx_add_sqr(s, a.c[2]);
-    return s;
+    return FxDot{{fx_get(s), fx_get(fx_sqr(a.c[2]))}, {2 * a.e[0], 2 * a.e[1]}};
 }
 
-// r.r as a double from sum 2^64 units of r^2 2^(58-2e): rounded to nearest.
-MH_HD double fx_square_to_double(FxSum sum, int e)
+MH_HD int fx_top(const FxDot &d) { return imax(d.e[0], d.e[1]); }
+
+// Its value in units of 2^(e-58), e >= fx_top.
+MH_HD long long fx_at(const FxDot &d, int e) { return sar(d.v[0], e - d.e[0]) + sar(d.v[1], e - d.e[1]); }
+
+// r.r as a double: rounded to nearest.
+MH_HD double fx_square_to_double(const FxDot &rr)
 {
-    unsigned long long u = (unsigned long long)fx_get_shl(sum, 4);      // r^2 2^(62-2e), below 2^64
+    const int e = fx_top(rr);
+    unsigned long long u = (unsigned long long)fx_at(rr, e) << 4;       // r^2 2^(62-e), below 2^64
     const int c = clz32((unsigned)(u >> 32));                           // 0 .. 3 unless r = 0
     u <<= c;
     unsigned long long b = (u >> 11) + ((unsigned)u >> 10 & 1u);
-    b += (unsigned long long)(unsigned)(1023 + 2 * e - c) << 52;        // the leading bit adds 1 to the exponent
+    b += (unsigned long long)(unsigned)(1023 + e - c) << 52;            // the leading bit adds 1 to the exponent
     if (c > 3) b = 0;
 #ifdef __CUDA_ARCH__
     return __longlong_as_double((long long)b);
@@ -288,10 +319,10 @@ struct FxBody {
 };
 
 // The powers s^-1 and s^(-3/2) and the terms of one pair with the differences
-// r^(k) = diff(k) = b^(k) - a^(k) (components c[c] 2^(e-61), the largest normalised).
+// r^(k) = diff(k) = b^(k) - a^(k) (components c[c] 2^(e-61), each group's largest normalised).
 // inverse(r, sinv, S): the FP64 powers of s = r.r + eps^2.  Calls weight(S) once, then
 // sink(k, A) for k = 0 .. P in order: A^(k)/(G m S) has components A.c[c] 2^(A.e-61),
-// the largest normalised.
+// each group's largest normalised.
 template <int P, typename Diff, typename Inverse, typename Weight, typename Sink>
 MH_HD void pair_terms(Diff &&diff, Inverse &&inverse, Weight &&weight, Sink &&sink)
 {
@@ -304,27 +335,37 @@ MH_HD void pair_terms(Diff &&diff, Inverse &&inverse, Weight &&weight, Sink &&si
     sink(0, r);
 
     const Fx3 v = diff(1);
-    const Fx rv = fx(fx_get_shl(fx_dot(r, v), 1));              // r.v 2^(59-er-ev)
-    long long an = fx_get_shl(fx_mul(rv, sinv), 3);             // alpha 2^(58-er-ev-q)
-    const int ea_ = r.e + v.e + q + 3 - fx_norm(an);            // alpha = an 2^(ea_-61)
+    const FxDot rvd = fx_dot(r, v);
+    const int erv = fx_top(rvd);
+    const Fx rv = fx((long long)((unsigned long long)fx_at(rvd, erv) << 1));   // r.v 2^(59-erv)
+    long long an = fx_get_shl(fx_mul(rv, sinv), 3);             // alpha 2^(58-erv-q)
+    const int ea_ = erv + q + 3 - fx_norm(an);                  // alpha = an 2^(ea_-61)
     const long long m3a = -(an + 2 * an);
     const Fx al = fx(an);
     {
-        const int e1 = imax(v.e, ea_ + 2 + r.e);
-        const Fx k1 = fx(sar(m3a, e1 - r.e - ea_));
-        const int nv = 3 + e1 - v.e;
         long long A[3];
+        int e[2];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-        for (int c = 0; c < 3; ++c) A[c] = fx_get(fx_mul(k1, r.c[c])) + sar(fx_val(v.c[c]), nv);
-        sink(1, fx_norm3(A, e1));
+        for (int g = 0; g < 2; ++g) {
+            e[g] = imax(v.e[g], ea_ + 2 + r.e[g]);
+            const Fx k1 = fx(sar(m3a, e[g] - r.e[g] - ea_));
+            const int nv = 3 + e[g] - v.e[g];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+            for (int c = fx_first(g); c < fx_first(g + 1); ++c)
+                A[c] = fx_get(fx_mul(k1, r.c[c])) + sar(fx_val(v.c[c]), nv);
+        }
+        sink(1, fx_norm3(A, e));
     }
     if constexpr (P >= 2) {
         const Fx3 w = diff(2);
         // v.v + r.a on the larger exponent of the two, times 1/s
-        const int eq = imax(2 * v.e, r.e + w.e);
-        const Fx vq = fx(sar(fx_get(fx_dot_self(v)), eq - 2 * v.e) + sar(fx_get(fx_dot(r, w)), eq - r.e - w.e));
+        const FxDot vv = fx_dot_self(v), rw = fx_dot(r, w);
+        const int eq = imax(fx_top(vv), fx_top(rw));
+        const Fx vq = fx(fx_at(vv, eq) + fx_at(rw, eq));
         const long long u0 = fx_get_shl(fx_mul(vq, sinv), 3);   // u 2^(57-eq-q)
         const long long p0 = fx_get_shl(fx_sqr(al), 2);         // alpha^2 2^(60-2 ea_)
         const int pu = eq + q - 57, pa = 2 * ea_ - 60;
@@ -334,26 +375,33 @@ MH_HD void pair_terms(Diff &&diff, Inverse &&inverse, Weight &&weight, Sink &&si
         const int ec2 = eu + 61 - fx_norm(m2);
         const long long m2x3 = m2 + 2 * m2;
         {
-            const int e2 = imax(w.e, imax(ea_ + 3 + v.e, ec2 + 2 + r.e));
-            const Fx k1 = fx(sar(m3a, e2 - v.e - ea_ - 1));
-            const Fx k2 = fx(sar(m2x3, e2 - r.e - ec2));
-            const int nw = 3 + e2 - w.e;
             long long A[3];
+            int e[2];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-            for (int c = 0; c < 3; ++c) {
-                FxSum t = fx_mul(k1, v.c[c]);
-                fx_add(t, k2, r.c[c]);
-                A[c] = fx_get(t) + sar(fx_val(w.c[c]), nw);
+            for (int g = 0; g < 2; ++g) {
+                e[g] = imax(w.e[g], imax(ea_ + 3 + v.e[g], ec2 + 2 + r.e[g]));
+                const Fx k1 = fx(sar(m3a, e[g] - v.e[g] - ea_ - 1));
+                const Fx k2 = fx(sar(m2x3, e[g] - r.e[g] - ec2));
+                const int nw = 3 + e[g] - w.e[g];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+                for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
+                    FxSum t = fx_mul(k1, v.c[c]);
+                    fx_add(t, k2, r.c[c]);
+                    A[c] = fx_get(t) + sar(fx_val(w.c[c]), nw);
+                }
             }
-            sink(2, fx_norm3(A, e2));
+            sink(2, fx_norm3(A, e));
         }
         if constexpr (P >= 3) {
             const Fx3 y = diff(3);
-            const int ez = imax(v.e + w.e, r.e + y.e);
-            const long long va = sar(fx_get(fx_dot(v, w)), ez - v.e - w.e);
-            const Fx zz = fx(va + 2 * va + sar(fx_get(fx_dot(r, y)), ez - r.e - y.e));
+            const FxDot vw = fx_dot(v, w), ry = fx_dot(r, y);
+            const int ez = imax(fx_top(vw), fx_top(ry));
+            const long long va = fx_at(vw, ez);
+            const Fx zz = fx(va + 2 * va + fx_at(ry, ez));
             const long long z0 = fx_get_shl(fx_mul(zz, sinv), 2);      // z 2^(56-ez-q)
             long long h = u + 2 * u - (8 * p - p);                     // (3 u - 7 alpha^2) 2^-eu
             const int eh = eu + 61 - fx_norm(h);
@@ -363,35 +411,41 @@ MH_HD void pair_terms(Diff &&diff, Inverse &&inverse, Weight &&weight, Sink &&si
             const long long t = sar(t0, et - pt);
             long long m3 = t + 4 * t - sar(z0, et - pz);               // (5 alpha h - z) 2^-et
             const int ec3 = et + 61 - fx_norm(m3);
-            const int e3 = imax(imax(y.e, ea_ + 4 + w.e), imax(ec2 + 4 + v.e, ec3 + 2 + r.e));
-            const Fx k1 = fx(sar(3 * (m3a >> 2), e3 - w.e - ea_ - 2));
-            const Fx k2 = fx(sar(3 * (m2x3 >> 2), e3 - v.e - ec2 - 2));
-            const Fx k3 = fx(sar(m3 + 2 * m3, e3 - r.e - ec3));
-            const int ny = 3 + e3 - y.e;
             long long A[3];
+            int e[2];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-            for (int c = 0; c < 3; ++c) {
-                FxSum s = fx_mul(k1, w.c[c]);
-                fx_add(s, k2, v.c[c]);
-                fx_add(s, k3, r.c[c]);
-                A[c] = fx_get(s) + sar(fx_val(y.c[c]), ny);
+            for (int g = 0; g < 2; ++g) {
+                e[g] = imax(imax(y.e[g], ea_ + 4 + w.e[g]), imax(ec2 + 4 + v.e[g], ec3 + 2 + r.e[g]));
+                const Fx k1 = fx(sar(3 * (m3a >> 2), e[g] - w.e[g] - ea_ - 2));
+                const Fx k2 = fx(sar(3 * (m2x3 >> 2), e[g] - v.e[g] - ec2 - 2));
+                const Fx k3 = fx(sar(m3 + 2 * m3, e[g] - r.e[g] - ec3));
+                const int ny = 3 + e[g] - y.e[g];
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+                for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
+                    FxSum s = fx_mul(k1, w.c[c]);
+                    fx_add(s, k2, v.c[c]);
+                    fx_add(s, k3, r.c[c]);
+                    A[c] = fx_get(s) + sar(fx_val(y.c[c]), ny);
+                }
             }
-            sink(3, fx_norm3(A, e3));
+            sink(3, fx_norm3(A, e));
         }
     }
 }
 
-// One pair of two bodies on the rows' grids E.  weight(MS, qS): S = MS 2^(qS-60);
-// rinv3(s, sinv, S): the FP64 powers of s.
+// One pair of two bodies on the rows' grids, E for the first two components and E + dz
+// for the third.  weight(MS, qS): S = MS 2^(qS-60); rinv3(s, sinv, S): the FP64 powers of s.
 template <int P, typename Rsqrt, typename Weight, typename Sink>
-MH_HD void pair_fix(const FxBody<P> &a, const FxBody<P> &b, const int (&E)[4], double eps2, Rsqrt &&rinv3,
+MH_HD void pair_fix(const FxBody<P> &a, const FxBody<P> &b, const int (&E)[4], int dz, double eps2, Rsqrt &&rinv3,
                     Weight &&weight, Sink &&sink)
 {
-    pair_terms<P>([&](int k) { return fx_diff(b.w[k], a.w[k], E[k]); },
+    pair_terms<P>([&](int k) { return fx_diff(b.w[k], a.w[k], E[k], E[k] + dz); },
                   [&](const Fx3 &r, double &sinv, double &S) {
-                      rinv3(fx_square_to_double(fx_dot_self(r), r.e) + eps2, sinv, S);
+                      rinv3(fx_square_to_double(fx_dot_self(r)) + eps2, sinv, S);
                   },
                   [&](double S) {
                       int qS;
