@@ -72,7 +72,7 @@ TRAFFIC = {"files": ["paper_2006_02501_gb300/csrc/pair_fix.cu",
            "sha256": [
                "7d479842edd11e0c7ccca49b62491923e2bfb2f01cef41efef89ba2b6c20e5b8",
                "c802ddbf2bc01bbe166b68cc004187b2551ec183e6bee6cd6593fc8650998fd6",
-               "d8ec6193aab9c24134d5972007fc7963475e8f2ecac408a8e0f0a8549176ff7e",
+               "bd815772c279aa4a52bf11ec15412676316dbd28c88ce200337303822d50c997",
                "1f0598f969a1334d8da9f876f87927fc5e369136c5e96fd84acba341d9b6ca6c"],
            # profiles/k_pair_fix_sym_disc_order8.md: 16.30 MB read + 40.29 MB written
            "bytes_per_launch": 16.30e6 + 40.29e6,

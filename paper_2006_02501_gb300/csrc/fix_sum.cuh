@@ -39,7 +39,8 @@ constexpr float kGapFlat = 2.2f;
 // (multiplicative hashing by the golden ratio).
 __device__ __forceinline__ int64_t fix_partner(int64_t i, int64_t N)
 {
-    return (i + 1 + (int64_t)__umulhi((unsigned)i * 2654435761u, (unsigned)(N - 1))) % N;
+    const int64_t j = i + 1 + (int64_t)__umulhi((unsigned)i * 2654435761u, (unsigned)(N - 1));
+    return j < N ? j : j - N;
 }
 
 // Gaps of a difference's components below the largest, axis `skip` left out.
