@@ -70,9 +70,9 @@ TRAFFIC = {"files": ["paper_2006_02501_gb300/csrc/pair_fix.cu",
                      "paper_2006_02501_gb300/csrc/fix_sum.cuh",
                      "paper_2006_02501_gb300/csrc/pair_sym.cuh"],
            "sha256": [
-               "7d479842edd11e0c7ccca49b62491923e2bfb2f01cef41efef89ba2b6c20e5b8",
+               "c58e7657a0d5115da3acba8b3d4db70e44fb0173c307813b5da94038198f9028",
                "c802ddbf2bc01bbe166b68cc004187b2551ec183e6bee6cd6593fc8650998fd6",
-               "bd815772c279aa4a52bf11ec15412676316dbd28c88ce200337303822d50c997",
+               "276682cd6ae64d40b6397df1b410f9ef54b7b982b922f0391e9438b52a932352",
                "1f0598f969a1334d8da9f876f87927fc5e369136c5e96fd84acba341d9b6ca6c"],
            # profiles/k_pair_fix_sym_disc_order8.md: 16.30 MB read + 40.29 MB written
            "bytes_per_launch": 16.30e6 + 40.29e6,
@@ -86,14 +86,18 @@ TRAFFIC = {"files": ["paper_2006_02501_gb300/csrc/pair_fix.cu",
 DD_INSTR = {"files": ["paper_2006_02501_gb300/csrc/dd.cu",
                       "paper_2006_02501_gb300/csrc/dd.cuh",
                       "paper_2006_02501_gb300/csrc/dd_fix.cuh",
-                      "paper_2006_02501_gb300/csrc/dd_pair_fix.cuh"],
-            "sha256": ["0d1035891afd1b9add13028b31ba489fbc37b8eacf5ecf586626250babbd5b6c",
+                      "paper_2006_02501_gb300/csrc/dd_pair_fix.cuh",
+                      "paper_2006_02501_gb300/csrc/pair_fix.cuh",
+                      "paper_2006_02501_gb300/csrc/fix_sum.cuh"],
+            "sha256": ["f75150ae70030496e86f67fe9a4d997a3695cc154267785a28c76f3416a7f9e3",
                        "f43f2591663c27103bf9ee43e6dda962e4fc0d99eef95b3953edd99ba0cb6c9a",
-                       "d49242dd496e153edb66ac56be60d429f64f977a2bae3f3f04b81433a78f86ce",
-                       "76886d2c956897b16b924f6ecfc20b159005dc77e5751ebdcd58438e634453c8"],
+                       "0301814481ee15e45def4e352642731e8d24a663393545655b5b898359bae7ad",
+                       "8161f09f51fe2d54f75d7e7308f46786ec1ca6b578338058d6f4e7498ff7d5c3",
+                       "c802ddbf2bc01bbe166b68cc004187b2551ec183e6bee6cd6593fc8650998fd6",
+                       "276682cd6ae64d40b6397df1b410f9ef54b7b982b922f0391e9438b52a932352"],
             # profiles/k_ddx_pair_sym_disc_N4096_order8.md: 137.2e6 FP64 thread and
-            # 662.3e6 ALU warp instructions for 4096 x 4095 pair interactions
-            "fp64_thread_instr_per_interaction": 8.18, "alu_thread_instr_per_interaction": 1263.0}
+            # 792.7e6 ALU warp instructions for 4096 x 4095 pair interactions
+            "fp64_thread_instr_per_interaction": 8.18, "alu_thread_instr_per_interaction": 1512.0}
 FP64_LANE_INSTR_PER_S = N_SM * 2 * SM_MAX_MHZ * 1e6
 
 

@@ -851,7 +851,7 @@ struct DDBatchDev {
 };
 
 // Records and header of the integer evaluation (P = 1 .. 3, one system): rec
-// ddx_rec_bytes(N), hdr ddx_hdr_bytes(N), its first 16 words zero before the
+// ddx_rec_bytes(N), hdr ddx_hdr_bytes(N), its first 24 words zero before the
 // first launch.
 struct DDxBuf {
     uint4 *rec = nullptr;

@@ -17,11 +17,12 @@
 // good to 2^-104 .. 2^-106.
 //
 // Inputs.  The components of a body's x, v, a, a-dot are 160-bit two's complement
-// integers on units of 2^(e-155) with an exponent e per vector (a and a-dot of
-// the bodies of a planetary system span 2^100).  Of two bodies the smaller vector is
-// shifted to the larger's unit, and the difference takes its exponent from its
-// leading bit: bits are lost only below 2^-153 of a difference that did not cancel.
-// The formulas are those of pair_fix.cuh.
+// integers on units of 2^(e-155) with an exponent e per vector and group of
+// components (a and a-dot of the bodies of a planetary system span 2^100).  Of two
+// bodies the smaller vector is shifted to the larger's unit, and the difference takes
+// its exponent from its leading bit: bits are lost only below 2^-153 of a difference
+// that did not cancel.  The formulas are those of pair_fix.cuh, and so are the groups:
+// the flattest axis of a system, its third component, has exponents of its own.
 #pragma once
 
 #include "pair_fix.cuh"
@@ -222,7 +223,7 @@ MH_HD int lx_norm(Lx &a)
 
 struct Lx3 {
     Lx c[3];
-    int e;
+    int e[2];          // of the first two components together and of the third
 };
 
 MH_HD unsigned shr32(unsigned lo, unsigned hi, int n)     // low word of (hi:lo) >> n, 0 <= n < 32
@@ -252,12 +253,16 @@ MH_HD void sub160(const unsigned (&a)[5], const unsigned (&b)[5], unsigned (&d)[
 #endif
 }
 
-// Vector words w >> n with sign, n >= 0.
+// Words of group g of a vector, w >> n with sign, n >= 0.
+template <int g>
 MH_HD void lx_shift_words(unsigned (&w)[3][5], int n)
 {
     n = imin(n, 159);
     while (n >= 32) {
-        for (int c = 0; c < 3; ++c) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
             w[c][0] = w[c][1];
             w[c][1] = w[c][2];
             w[c][2] = w[c][3];
@@ -269,51 +274,46 @@ MH_HD void lx_shift_words(unsigned (&w)[3][5], int n)
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-    for (int c = 0; c < 3; ++c) {
+    for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
         for (int k = 0; k < 4; ++k) w[c][k] = shr32(w[c][k], w[c][k + 1], n);
         w[c][4] = (unsigned)((int)w[c][4] >> n);
     }
 }
 
-// b - a: words of unit 2^(eb-155) and 2^(ea-155).
-MH_HD Lx3 lx_diff(const unsigned (&bw)[3][5], int eb, const unsigned (&aw)[3][5], int ea)
+// Group g of b - a: words of unit 2^(eb-155) and 2^(ea-155).
+template <int g>
+MH_HD void lx_diff_group(unsigned (&b)[3][5], int eb, unsigned (&a)[3][5], int ea, Lx3 &r)
 {
-    unsigned a[3][5], b[3][5], d[3][5];
-    for (int c = 0; c < 3; ++c)
-        for (int k = 0; k < 5; ++k) {
-            a[c][k] = aw[c][k];
-            b[c][k] = bw[c][k];
-        }
-    if (ea < eb) lx_shift_words(a, eb - ea);
-    if (eb < ea) lx_shift_words(b, ea - eb);
-    const int E = imax(ea, eb);
+    unsigned d[3][5];
+    if (ea < eb) lx_shift_words<g>(a, eb - ea);
+    if (eb < ea) lx_shift_words<g>(b, ea - eb);
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-    for (int c = 0; c < 3; ++c) sub160(b[c], a[c], d[c]);
-    auto fold = [&]() {
-        return (d[0][4] ^ d[0][4] + d[0][4]) | (d[1][4] ^ d[1][4] + d[1][4]) | (d[2][4] ^ d[2][4] + d[2][4]);
-    };
+    for (int c = fx_first(g); c < fx_first(g + 1); ++c) sub160(b[c], a[c], d[c]);
+    auto fold = [&]() { return g ? fold1(d[2][4]) : fold1(d[0][4]) | fold1(d[1][4]); };
     unsigned t = fold();
-    Lx3 r;
-    r.e = E + 2;
+    int e = imax(ea, eb) + 2;
     for (int k = 0; k < 5 && t < 2; ++k) {
-        for (int c = 0; c < 3; ++c) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
             d[c][4] = shl32(d[c][3], d[c][4], 29);
             d[c][3] = shl32(d[c][2], d[c][3], 29);
             d[c][2] = shl32(d[c][1], d[c][2], 29);
             d[c][1] = shl32(d[c][0], d[c][1], 29);
             d[c][0] <<= 29;
         }
-        r.e -= 29;
+        e -= 29;
         t = fold();
     }
     const int n = imin(clz32(t), 31) - 2;              // top word's magnitude to [2^28, 2^29)
-    r.e -= n;
+    r.e[g] = e - n;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-    for (int c = 0; c < 3; ++c) {
+    for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
         const unsigned w4 = shl32(d[c][3], d[c][4], n), w3 = shl32(d[c][2], d[c][3], n);
         const unsigned w2 = shl32(d[c][1], d[c][2], n), w1 = shl32(d[c][0], d[c][1], n);
         // mantissa = bits 46 .. 157
@@ -322,45 +322,89 @@ MH_HD Lx3 lx_diff(const unsigned (&bw)[3][5], int eb, const unsigned (&aw)[3][5]
         r.c[c].l[2] = (int)((w3 >> 6 | w4 << 26) & (unsigned)kLmask);
         r.c[c].l[3] = (int)w4 >> 2;
     }
+}
+
+MH_HD Lx3 lx_diff(const unsigned (&bw)[3][5], const int (&eb)[2], const unsigned (&aw)[3][5], const int (&ea)[2])
+{
+    unsigned a[3][5], b[3][5];
+    for (int c = 0; c < 3; ++c)
+        for (int k = 0; k < 5; ++k) {
+            a[c][k] = aw[c][k];
+            b[c][k] = bw[c][k];
+        }
+    Lx3 r;
+    lx_diff_group<0>(b, eb[0], a, ea[0], r);
+    lx_diff_group<1>(b, eb[1], a, ea[1], r);
     return r;
 }
 
-MH_HD LxSum lx_dot(const Lx3 &a, const Lx3 &b)
+// a.b as v[0] 2^(e[0]-110) + v[1] 2^(e[1]-110), |v[0]| <= 2^111, |v[1]| <= 2^110.
+struct LxDot {
+    Lx v[2];
+    int e[2];
+};
+
+MH_HD LxDot lx_dot(const Lx3 &a, const Lx3 &b)
 {
-    LxSum s = lx_zero();
+    LxSum s = lx_zero(), z = lx_zero();
     lx_add(s, a.c[0], b.c[0]);
     lx_add(s, a.c[1], b.c[1]);
-    lx_add(s, a.c[2], b.c[2]);
-    return s;
+    lx_add(z, a.c[2], b.c[2]);
+    return LxDot{{lx_get(s), lx_get(z)}, {a.e[0] + b.e[0], a.e[1] + b.e[1]}};
 }
 
-// Three components v 2^(e-110), normalised together.
-MH_HD Lx3 lx_norm3(const Lx (&v)[3], int e)
+MH_HD LxDot lx_dot_self(const Lx3 &a)
 {
-    Lx3 r;
-    r.c[0] = v[0];
-    r.c[1] = v[1];
-    r.c[2] = v[2];
-    r.e = e + 1;
-    auto fold = [&]() { return lx_top(r.c[0].l[3]) | lx_top(r.c[1].l[3]) | lx_top(r.c[2].l[3]); };
+    LxSum s = lx_zero(), z = lx_zero();
+    lx_add_sqr(s, a.c[0]);
+    lx_add_sqr(s, a.c[1]);
+    lx_add_sqr(z, a.c[2]);
+    return LxDot{{lx_get(s), lx_get(z)}, {2 * a.e[0], 2 * a.e[1]}};
+}
+
+MH_HD int lx_upper(const LxDot &d) { return imax(d.e[0], d.e[1]); }
+
+// Its value in units of 2^(e-110), e >= lx_upper.
+MH_HD Lx lx_at(const LxDot &d, int e) { return lx_plus(lx_sar(d.v[0], e - d.e[0]), lx_sar(d.v[1], e - d.e[1])); }
+
+// Group g of the components v 2^(e-110), normalised.
+template <int g>
+MH_HD void lx_norm_group(const Lx (&v)[3], int e, Lx3 &r)
+{
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+    for (int c = fx_first(g); c < fx_first(g + 1); ++c) r.c[c] = v[c];
+    e += 1;
+    auto fold = [&]() { return g ? lx_top(r.c[2].l[3]) : lx_top(r.c[0].l[3]) | lx_top(r.c[1].l[3]); };
     unsigned t = fold();
     for (int k = 0; k < 3 && t < 2; ++k) {
-        for (int c = 0; c < 3; ++c) {
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+        for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
             Lx &a = r.c[c];
             a.l[3] = (int)((unsigned)a.l[3] << kLb) | a.l[2];
             a.l[2] = a.l[1];
             a.l[1] = a.l[0];
             a.l[0] = 0;
         }
-        r.e -= kLb;
+        e -= kLb;
         t = fold();
     }
     const int b = imin(clz32(t), 31) - 4;
-    r.e -= b;
+    r.e[g] = e - b;
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-    for (int c = 0; c < 3; ++c) r.c[c] = b >= 0 ? lx_shl(r.c[c], b) : lx_sar(r.c[c], -b);
+    for (int c = fx_first(g); c < fx_first(g + 1); ++c) r.c[c] = b >= 0 ? lx_shl(r.c[c], b) : lx_sar(r.c[c], -b);
+}
+
+MH_HD Lx3 lx_norm3(const Lx (&v)[3], const int (&e)[2])
+{
+    Lx3 r;
+    lx_norm_group<0>(v, e[0], r);
+    lx_norm_group<1>(v, e[1], r);
     return r;
 }
 
@@ -373,14 +417,15 @@ struct LxNum {
 constexpr int kLxZero = -20000;        // exponent of the representation of zero
 constexpr int kLxBad = 1 << 24;        // exponent of S for s = 0
 
-// s = r.r + eps^2 from the sum of squares (r.r = get 2^(2e-110)); s^-1 and s^(-3/2).
+// s = r.r + eps^2; s^-1 and s^(-3/2).
 // rsqrt(f): 1/sqrt(f) in FP64, f in [0.5, 2).  One third-order step from it:
 // y = y0 (1 + d/2 + 3 d^2/8), d = 1 - f y0^2 ~ 2^-52, f y0^2 to 2^-111.
 template <typename Rsqrt>
-MH_HD void lx_inverse(const LxSum &rr, int re, const LxNum &eps2, Rsqrt &&rsqrt, LxNum &sinv, LxNum &S)
+MH_HD void lx_inverse(const LxDot &rr, const LxNum &eps2, Rsqrt &&rsqrt, LxNum &sinv, LxNum &S)
 {
-    Lx s = lx_get(rr);
-    int es = 2 * re + 1;
+    int es = lx_upper(rr);
+    Lx s = lx_at(rr, es);
+    es += 1;
     es -= lx_norm(s);                                  // s 2^(es-111)
     if ((s.l[1] | s.l[2] | s.l[3]) == 0) es = kLxZero;  // (l0 may hold the rounding of a zero sum)
     if (eps2.e > kLxZero) {
@@ -434,7 +479,7 @@ MH_HD void lx_inverse(const LxSum &rr, int re, const LxNum &eps2, Rsqrt &&rsqrt,
 template <int P>
 struct LxBody {
     unsigned w[P + 1][3][5];
-    int e[P + 1];
+    int e[P + 1][2];
 };
 
 // One pair: r^(k) = b^(k) - a^(k), as pair_fix.  weight(S) once, then sink(k, A) for
@@ -445,11 +490,7 @@ MH_HD void pair_wide(const LxBody<P> &a, const LxBody<P> &b, const LxNum &eps2, 
 {
     const Lx3 r = lx_diff(b.w[0], b.e[0], a.w[0], a.e[0]);
     LxNum sinv, S;
-    {
-        LxSum rr = lx_zero();
-        for (int c = 0; c < 3; ++c) lx_add_sqr(rr, r.c[c]);
-        lx_inverse(rr, r.e, eps2, rsqrt, sinv, S);
-    }
+    lx_inverse(lx_dot_self(r), eps2, rsqrt, sinv, S);
     const int q = sinv.e;
     weight(S);
     sink(0, r);
@@ -457,27 +498,40 @@ MH_HD void pair_wide(const LxBody<P> &a, const LxBody<P> &b, const LxNum &eps2, 
     const Lx3 v = lx_diff(b.w[1], b.e[1], a.w[1], a.e[1]);
     // products of scalars carry a factor of 2: their rounding reaches a^(3) times 7 and 5
     const Lx sv = lx_twice(sinv.m);
-    Lx an = lx_mul(lx_get(lx_dot(r, v)), sv);                  // alpha 2^(110-er-ev-q)
-    const int ea_ = r.e + v.e + q + 1 - lx_norm(an);           // alpha = an 2^(ea_-111)
+    Lx an;
+    int ea_;
+    {
+        const LxDot rv = lx_dot(r, v);
+        const int erv = lx_upper(rv);
+        an = lx_mul(lx_at(rv, erv), sv);                       // alpha 2^(110-erv-q)
+        ea_ = erv + q + 1 - lx_norm(an);                       // alpha = an 2^(ea_-111)
+    }
     const Lx m3a = lx_scale(-3, an);
     {
-        const int e1 = imax(v.e, ea_ + 2 + r.e);
-        const Lx k1 = lx_sar(m3a, e1 - r.e - ea_);
         Lx A[3];
+        int e[2];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-        for (int c = 0; c < 3; ++c) A[c] = lx_plus(lx_mul(k1, r.c[c]), lx_sar(v.c[c], 1 + e1 - v.e));
-        sink(1, lx_norm3(A, e1));
+        for (int g = 0; g < 2; ++g) {
+            e[g] = imax(v.e[g], ea_ + 2 + r.e[g]);
+            const Lx k1 = lx_sar(m3a, e[g] - r.e[g] - ea_);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+            for (int c = fx_first(g); c < fx_first(g + 1); ++c)
+                A[c] = lx_plus(lx_mul(k1, r.c[c]), lx_sar(v.c[c], 1 + e[g] - v.e[g]));
+        }
+        sink(1, lx_norm3(A, e));
     }
     if constexpr (P >= 2) {
         const Lx3 w = lx_diff(b.w[2], b.e[2], a.w[2], a.e[2]);
-        const int eq = imax(2 * v.e, r.e + w.e);
+        int eq;
         Lx vv;
         {
-            LxSum t = lx_zero();
-            for (int c = 0; c < 3; ++c) lx_add_sqr(t, v.c[c]);
-            vv = lx_plus(lx_sar(lx_get(t), eq - 2 * v.e), lx_sar(lx_get(lx_dot(r, w)), eq - r.e - w.e));
+            const LxDot v2 = lx_dot_self(v), rw = lx_dot(r, w);
+            eq = imax(lx_upper(v2), lx_upper(rw));
+            vv = lx_plus(lx_at(v2, eq), lx_at(rw, eq));
         }
         const Lx a2 = lx_twice(an);
         const Lx u0 = lx_mul(vv, sv);                          // u 2^(110-eq-q), below 3 2^111
@@ -488,26 +542,36 @@ MH_HD void pair_wide(const LxBody<P> &a, const LxBody<P> &b, const LxNum &eps2, 
         Lx m2 = lx_comb(5, p, -1, u);
         const int ec2 = eu + 111 - lx_norm(m2);
         {
-            const int e2 = imax(w.e, imax(ea_ + 3 + v.e, ec2 + 2 + r.e));
-            const Lx k1 = lx_sar(m3a, e2 - v.e - ea_ - 1);
-            const Lx k2 = lx_sar(lx_scale(3, m2), e2 - r.e - ec2);
             Lx A[3];
+            int e[2];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-            for (int c = 0; c < 3; ++c) {
-                LxSum t = lx_zero();
-                lx_add(t, k1, v.c[c]);
-                lx_add(t, k2, r.c[c]);
-                A[c] = lx_plus(lx_get(t), lx_sar(w.c[c], 1 + e2 - w.e));
+            for (int g = 0; g < 2; ++g) {
+                e[g] = imax(w.e[g], imax(ea_ + 3 + v.e[g], ec2 + 2 + r.e[g]));
+                const Lx k1 = lx_sar(m3a, e[g] - v.e[g] - ea_ - 1);
+                const Lx k2 = lx_sar(lx_scale(3, m2), e[g] - r.e[g] - ec2);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+                for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
+                    LxSum t = lx_zero();
+                    lx_add(t, k1, v.c[c]);
+                    lx_add(t, k2, r.c[c]);
+                    A[c] = lx_plus(lx_get(t), lx_sar(w.c[c], 1 + e[g] - w.e[g]));
+                }
             }
-            sink(2, lx_norm3(A, e2));
+            sink(2, lx_norm3(A, e));
         }
         if constexpr (P >= 3) {
             const Lx3 y = lx_diff(b.w[3], b.e[3], a.w[3], a.e[3]);
-            const int ez = imax(v.e + w.e, r.e + y.e);
-            const Lx zz = lx_comb(3, lx_sar(lx_get(lx_dot(v, w)), ez - v.e - w.e), 1,
-                                  lx_sar(lx_get(lx_dot(r, y)), ez - r.e - y.e));
+            int ez;
+            Lx zz;
+            {
+                const LxDot vw = lx_dot(v, w), ry = lx_dot(r, y);
+                ez = imax(lx_upper(vw), lx_upper(ry));
+                zz = lx_comb(3, lx_at(vw, ez), 1, lx_at(ry, ez));
+            }
             const Lx z0 = lx_mul(zz, sv);                      // z 2^(110-ez-q), below 3 2^112
             Lx h = lx_comb(3, u, -7, p);
             const int eh = eu + 111 - lx_norm(h);
@@ -516,22 +580,28 @@ MH_HD void pair_wide(const LxBody<P> &a, const LxBody<P> &b, const LxNum &eps2, 
             const int et = imax(pt, pz);
             Lx m3 = lx_comb(5, lx_sar_near(t0, et - pt), -1, lx_sar_near(z0, et - pz));
             const int ec3 = et + 111 - lx_norm(m3);
-            const int e3 = imax(imax(y.e, ea_ + 4 + w.e), imax(ec2 + 4 + v.e, ec3 + 2 + r.e));
-            const Lx k1 = lx_sar(lx_scale(-9, an), e3 - w.e - ea_);
-            const Lx k2 = lx_sar(lx_scale(9, m2), e3 - v.e - ec2);
-            const Lx k3 = lx_sar(lx_scale(3, m3), e3 - r.e - ec3);
             Lx A[3];
+            int e[2];
 #ifdef __CUDACC__
 #pragma unroll
 #endif
-            for (int c = 0; c < 3; ++c) {
-                LxSum t = lx_zero();
-                lx_add(t, k1, w.c[c]);
-                lx_add(t, k2, v.c[c]);
-                lx_add(t, k3, r.c[c]);
-                A[c] = lx_plus(lx_get(t), lx_sar(y.c[c], 1 + e3 - y.e));
+            for (int g = 0; g < 2; ++g) {
+                e[g] = imax(imax(y.e[g], ea_ + 4 + w.e[g]), imax(ec2 + 4 + v.e[g], ec3 + 2 + r.e[g]));
+                const Lx k1 = lx_sar(lx_scale(-9, an), e[g] - w.e[g] - ea_);
+                const Lx k2 = lx_sar(lx_scale(9, m2), e[g] - v.e[g] - ec2);
+                const Lx k3 = lx_sar(lx_scale(3, m3), e[g] - r.e[g] - ec3);
+#ifdef __CUDACC__
+#pragma unroll
+#endif
+                for (int c = fx_first(g); c < fx_first(g + 1); ++c) {
+                    LxSum t = lx_zero();
+                    lx_add(t, k1, w.c[c]);
+                    lx_add(t, k2, v.c[c]);
+                    lx_add(t, k3, r.c[c]);
+                    A[c] = lx_plus(lx_get(t), lx_sar(y.c[c], 1 + e[g] - y.e[g]));
+                }
             }
-            sink(3, lx_norm3(A, e3));
+            sink(3, lx_norm3(A, e));
         }
     }
 }

@@ -30,10 +30,12 @@ __device__ __forceinline__ int exponent_field(double x)
 // or one thick population among others, leaves the gaps of the rest in them.
 //
 // The flattest axis, by the smallest of its rows' means, takes the separate exponent of
-// Fx3.  Where the other two have a mean above kGapFlat between them (a gap of 2^-1.3 more
-// than a plane's own), what is smaller would be less exact than in FP64, which it then takes.
+// Fx3.  Where the other two have a mean above gap_limit between them (a bit more than a
+// plane's own, and a margin for the spread of n bodies' mean), what is smaller would be less
+// exact than in FP64, which it then takes.
 constexpr int kGapMax = 15;
-constexpr float kGapFlat = 2.2f;
+
+__device__ __forceinline__ float gap_limit(int64_t n) { return 2.0f + 6.0f * rsqrtf((float)n); }
 
 // The other body of the difference: i plus a step that spreads over the system
 // (multiplicative hashing by the golden ratio).
