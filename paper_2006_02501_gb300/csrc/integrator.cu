@@ -722,17 +722,26 @@ __global__ void k_init_reduce(int64_t N, int64_t ld, int nr, int lo, int hi, int
         }
 }
 
-// out rows [0, nr) <- sum over S slots (mh_pair_eval's reduction).
-__global__ void k_reduce_out(int64_t n, int64_t ld_part, int nr, int split, const double *part,
-                             double *out)
+// out rows [0, nr) <- sum over S slots in slot order (mh_pair_eval's reduction), one
+// thread per (row, body): plans of a few hundred bodies have up to a hundred slots, and
+// one thread per body added those of its 12 rows one load after another (725 bodies,
+// P = 3: the call 201 us, 86 us; 64 bodies from 8192 sources 693 us, 170 us).
+__global__ void k_reduce_out(int64_t n, int64_t ld_part, int nr, int split, const double *__restrict__ part,
+                             double *__restrict__ out)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int r = 0; r < nr; ++r) {
-        double s = 0.0;
-        for (int q = 0; q < split; ++q) s += part[((int64_t)q * nr + r) * ld_part + i];
-        out[r * n + i] = s;
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (int64_t)nr * n) return;
+    const int64_t r = e / n, i = e - r * n;
+    double s = 0.0;
+    for (int q0 = 0; q0 < split; q0 += 8) {
+        double b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) b[u] = q0 + u < split ? part[((int64_t)(q0 + u) * nr + r) * ld_part + i] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (q0 + u < split) s += b[u];
     }
+    out[e] = s;
 }
 
 // max |x| and max |v| over the bodies of FP64 SoA rows (stride N) into bound[0..1]
@@ -972,7 +981,7 @@ int launch_split32(int64_t N, int P, const double *traj, const double *m, double
 int launch_reduce_out(int64_t n, int64_t ld_part, int nr, int split, const double *part, double *out,
                       cudaStream_t st)
 {
-    k_reduce_out<<<blocks_for(n, 128), 128, 0, st>>>(n, ld_part, nr, split, part, out);
+    k_reduce_out<<<blocks_for(n * nr, 128), 128, 0, st>>>(n, ld_part, nr, split, part, out);
     MH_LAUNCHED("k_reduce_out");
     return MH_OK;
 }
