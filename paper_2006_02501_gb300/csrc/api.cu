@@ -251,7 +251,7 @@ int tuned_variant(mh_sim *sim, int P, int64_t n_i, const int *ilist, int *varian
 // Whether n_i bodies from n_j are evaluated in fixed point (ordered pairs).
 bool use_fix(int P, int precision, int64_t n_i, int64_t n_j)
 {
-    return precision == MH_PREC_FP64 && P <= 3 && n_i * n_j >= kFixMinPairs;
+    return precision == MH_PREC_FP64 && fix_pays(P, n_i, n_j);
 }
 
 // One O(N^2) evaluation of a^(0..P) for all bodies into s.part; returns S via *split.

@@ -2,7 +2,7 @@
 // ordered pair: the kernels for active lists (block steps), small systems,
 // the initialisation passes above P = 5, and mh_pair_eval.  Shared-step
 // evaluations of larger systems take the pair-symmetric kernels of pair_fix.cu
-// and pair_sym.cu instead, and FP64 evaluations of 2^19 pairs up with P <= 3 the
+// and pair_sym.cu instead, and larger FP64 evaluations with P <= 3 (fix_pays) the
 // fixed-point kernel of pair_fix.cu.
 //
 // Pair physics (Dittmann 2020, Section 3, intro): a_ij = G m_j r_ij s^(-3/2),
