@@ -263,7 +263,7 @@ __global__ void k_correct(StepArgs a)
             // convergence of P(EC)^n: largest change of a position component, and the scale
             double dx = 0.0, xm = 0.0;
             if (live) {
-                dx = fabs(x - a.x1[c * a.ld + i]);
+                dx = fmax(dx, fabs(x - a.x1[c * a.ld + i]));      // (a NaN is the flag's, not counted)
                 xm = fmax(xm, fabs(x));
             }
             if (!(dx <= 1e300)) dx = 1e300;
