@@ -70,7 +70,7 @@ TRAFFIC = {"files": ["paper_2006_02501_gb300/csrc/pair_fix.cu",
                      "paper_2006_02501_gb300/csrc/fix_sum.cuh",
                      "paper_2006_02501_gb300/csrc/pair_sym.cuh"],
            "sha256": [
-               "c58e7657a0d5115da3acba8b3d4db70e44fb0173c307813b5da94038198f9028",
+               "889118b4b56bc22564e80a436dcdec2035a1f498751b18e678ea550b7a4ce283",
                "c802ddbf2bc01bbe166b68cc004187b2551ec183e6bee6cd6593fc8650998fd6",
                "276682cd6ae64d40b6397df1b410f9ef54b7b982b922f0391e9438b52a932352",
                "1f0598f969a1334d8da9f876f87927fc5e369136c5e96fd84acba341d9b6ca6c"],
