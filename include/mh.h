@@ -265,7 +265,7 @@ int mh_batch_energy(mh_sim *sim, double *energy);
 /* derivative stacks N x 2p x 3 x 2, scalars 2 doubles.  Masses, eps, G and dt  */
 /* are doubles (exact inputs).  Pair terms of orders 4 to 8 are formed in      */
 /* 112-bit integer arithmetic of the same or smaller rounding.  The cost per   */
-/* pair is about 6 times that of the FP64 form (orders 10 and 12: 20 times):   */
+/* pair is about 7 times that of the FP64 form (orders 10 and 12: 20 times):   */
 /* the form is meant for systems of a few to a few thousand bodies.            */
 /* ------------------------------------------------------------------------- */
 

@@ -369,7 +369,8 @@ class DDSimulation:
 
     x, v: (N, 3) doubles or (N, 3, 2) (hi, lo) pairs.  Results come back as
     (..., 2) pairs; value = hi + lo.  symmetric: each unordered pair evaluated
-    once for both bodies (k_dd_pair_sym), 1 = from 2048 bodies up (default),
+    once for both bodies (k_ddx_pair_sym up to 8th order, k_dd_pair_sym above),
+    1 = from 2048 bodies up (default),
     2 = always, 0 = never.
     """
 

@@ -6,8 +6,8 @@
 // Every product is one GEMM kernel on the tensor cores, mma.sync m16n8k16 with
 // bf16 operands and fp32 accumulators; ldmatrix absorbs the transposes of the
 // backward pass, the epilogues bias, activation and its derivative.  Weight
-// gradients, sums over the batch, have a kernel of their own.  Elementwise kernels form the mean-squared-error gradient, sum bias
-// gradients and take the Adam step (Kingma & Ba 2015) on an FP32 master copy of
+// gradients, sums over the batch, have a kernel of their own.  Elementwise kernels form
+// the mean-squared-error gradient, sum bias gradients and take the Adam step (Kingma & Ba 2015) on an FP32 master copy of
 // the parameters, refreshed into bf16 after every step.
 #include <cuda_bf16.h>
 
@@ -170,12 +170,14 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K, const bf
 
 // Weight gradients C[M x N] = A^T B, sums over the batch of up to 2^24 rows: one
 // chain of products per output element in row order, as k_gemm_bf16 takes them
-// (the tensor core rounds each step towards zero, so cutting the chain changes a
-// gradient of 65537 rows by 7e-5).  The chain's latency is the bound, 16 rows a
-// step; small output tiles put it on as many SMs as there are tiles and the rows
-// come through a ring of asynchronous copies.  All weights of the network in one
-// launch: the gradients of 65537 rows took 8 ms each on one to four SMs with a
-// barrier and element-wise loads every 16 rows.
+// (the tensor core rounds each step towards zero, so cutting the chain changes the
+// weights' gradients of 65537 rows by 7e-5 of their size).  Small output tiles put the
+// chains on as many SMs as there are tiles and the rows come through a ring of
+// asynchronous copies.  Bound by the ring: ~630 cycles per 64-row stage, of which the
+// chain's four dependent products take 82 (20.4 each, measured); the rest is the
+// copies' latency with three stages in flight and a barrier per stage.  All weights of
+// the network in one launch: the gradients of 65537 rows took 8 ms each on one to four
+// SMs with a barrier and element-wise loads every 16 rows, 313 us now.
 constexpr int kWT = 32, kWK = 64, kWStages = 4;
 
 struct WGrad {
